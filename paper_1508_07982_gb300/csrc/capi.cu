@@ -1392,8 +1392,10 @@ lbm_status build_phases(lbm_batch* b) {
         for (int m = 0; m < ph.n; m++) std::fill(owner.begin() + hprefix[k][m], owner.begin() + hprefix[k][m + 1], m);
         lbm_status st;
         if ((st = upload(b->mem, &q.owner, owner)) || (st = upload(b->mem, &q.args[0], hargs[0][k])) || (st = upload(b->mem, &q.args[1], hargs[1][k])) ||
-            (st = upload(b->mem, &q.prefix, hprefix[k])))
+            (st = upload(b->mem, &q.prefix, hprefix[k]))) {
+            free_phases(b);   // a list that ends early would be taken for the whole step by the next call
             return st;
+        }
     }
     return LBM_OK;
 }
