@@ -703,11 +703,16 @@ lbm_status ensure_acts(lbm_net* n, long long N) {
     const size_t bytes = size_t(N) * CH * sizeof(__nv_bfloat16);
     for (int l = 0; l <= n->layers; l++) {
         __nv_bfloat16* p = nullptr;
-        if (!n->mem.get(&p, bytes)) return nfail(LBM_ENOMEM, "cannot allocate the activations");
+        if (!n->mem.get(&p, bytes)) {
+            free_acts(n);
+            return nfail(LBM_ENOMEM, "cannot allocate the activations");
+        }
         n->act.push_back(p);
     }
-    if (!n->mem.get(&n->g0, bytes) || !n->mem.get(&n->g1, bytes))
+    if (!n->mem.get(&n->g0, bytes) || !n->mem.get(&n->g1, bytes)) {
+        free_acts(n);
         return nfail(LBM_ENOMEM, "cannot allocate the activation gradients");
+    }
     n->cap = N;
     return LBM_OK;
 }
@@ -814,8 +819,10 @@ lbm_status check_dims(int D, int H, int W, int nvol, Dims& d) {
     return LBM_OK;
 }
 
-// Forward pass over x (BF16 [N][16]); keeps every layer's input for the backward pass.
+// Forward pass over x (BF16 [N][16]); keeps every layer's input for the backward pass.  n->d stays empty until every
+// layer is enqueued, so that no gradient follows a pass that was refused.
 lbm_status forward(lbm_net* n, const __nv_bfloat16* x, const Dims& d) {
+    n->d = Dims{};
     lbm_status s = ensure_acts(n, d.N);
     if (s) return s;
     // The copy of the input that a later gradient needs runs beside the layers (512 volumes of 18^3: 32 us, the
