@@ -666,7 +666,8 @@ struct lbm_net {
     cudaStream_t side = nullptr;           // the copy of the input beside the layers
     cudaEvent_t ev[2] = {nullptr, nullptr};
     float* params = nullptr;   // per layer: W [27][16][16], b [16]
-    float* grads = nullptr;
+    float* grads = nullptr;    // of the last gradient call that was accepted
+    float* gsum = nullptr;     // sums of the call at work; the two change places when it is accepted
     float* m = nullptr;
     float* v = nullptr;
     __nv_bfloat16* wf = nullptr;   // per layer: forward BF16 weights
@@ -889,7 +890,8 @@ lbm_status lbm_net_create(int32_t layers, int32_t in_channels, int32_t out_chann
         lbm::set_last_error(keep.c_str());
         return s;
     };
-    if (!n->mem.get(&n->params, np * 4) || !n->mem.get(&n->grads, np * 4) || !n->mem.get(&n->m, np * 4) ||
+    if (!n->mem.get(&n->params, np * 4) || !n->mem.get(&n->grads, np * 4) || !n->mem.get(&n->gsum, np * 4) ||
+        !n->mem.get(&n->m, np * 4) ||
         !n->mem.get(&n->v, np * 4) || !n->mem.get(&n->wf, size_t(layers) * TAPS * CH * CH * 2) ||
         !n->mem.get(&n->wb, size_t(layers) * TAPS * CH * CH * 2) || !n->mem.get(&n->d_st, sizeof(Status)) ||
         cudaMallocHost(&n->h_st, sizeof(Status)) != cudaSuccess)
@@ -916,7 +918,7 @@ lbm_status lbm_net_destroy(lbm_net* n) {
     if (n->stream) cudaStreamSynchronize(n->stream);
     free_acts(n);
     for (const void* p : {static_cast<const void*>(n->params), static_cast<const void*>(n->grads),
-                          static_cast<const void*>(n->m), static_cast<const void*>(n->v),
+                          static_cast<const void*>(n->gsum), static_cast<const void*>(n->m), static_cast<const void*>(n->v),
                           static_cast<const void*>(n->wf), static_cast<const void*>(n->wb),
                           static_cast<const void*>(n->d_st)})
         n->mem.put(p);
@@ -992,7 +994,7 @@ lbm_status lbm_net_gradient(lbm_net* n, const float* skip, const float* target, 
     const Dims& d = n->d;
     // the sum of the weights stays on the device until the loss is read (the MSE denominator is nout times it)
     NCU(cudaMemsetAsync(n->d_st, 0, offsetof(Status, err), n->stream));
-    NCU(cudaMemsetAsync(n->grads, 0, size_t(n->layers) * PER_LAYER * 4, n->stream));
+    NCU(cudaMemsetAsync(n->gsum, 0, size_t(n->layers) * PER_LAYER * 4, n->stream));
     if (weight) {
         weight_sum_kernel<<<int(std::min<long long>((d.N + 255) / 256, 2LL * n->sms)), 256, 0, n->stream>>>(weight, d.N, n->d_st);
     } else {
@@ -1014,7 +1016,7 @@ lbm_status lbm_net_gradient(lbm_net* n, const float* skip, const float* target, 
     for (int l = n->layers - 1; l >= 0 && !cs; l--) {
         NCU(cudaEventRecord(n->ev[0], n->stream));
         NCU(cudaStreamWaitEvent(n->side, n->ev[0], 0));
-        wgrad_kernel<<<wgrid, kWgradThreads, g.smem, n->side>>>(n->act[l], dz, n->grads + size_t(l) * PER_LAYER, d, g);
+        wgrad_kernel<<<wgrid, kWgradThreads, g.smem, n->side>>>(n->act[l], dz, n->gsum + size_t(l) * PER_LAYER, d, g);
         if (l > 0) {
             cs = conv(n, dz, n->wb + size_t(l) * TAPS * CH * CH, nullptr, dx, d, 2, n->act[l]);
             std::swap(dz, dx);
@@ -1026,9 +1028,12 @@ lbm_status lbm_net_gradient(lbm_net* n, const float* skip, const float* target, 
     NCU(cudaGetLastError());
     const lbm_status st = check_err(n);
     const double count = n->h_st->weights * n->cout;
-    if (!st && !(count > 0.0)) return nfail(LBM_EINVAL, "the loss weights are all zero");
-    if (!st && loss) *loss = n->h_st->loss / count;
-    return st;
+    if (st) return st;
+    // known only now, after sums over NaN (the loss divides by the count): they are not published
+    if (!(count > 0.0)) return nfail(LBM_EINVAL, "the loss weights are all zero");
+    std::swap(n->grads, n->gsum);
+    if (loss) *loss = n->h_st->loss / count;
+    return LBM_OK;
 }
 
 lbm_status lbm_net_set_wait_test(lbm_net* n, int32_t on) {

@@ -1,4 +1,5 @@
-"""Net calls that are refused: a forward pass whose activations cannot be allocated."""
+"""Net calls that are refused: a forward pass whose activations cannot be allocated, loss weights without a positive
+sum, a tensor-core wait that runs out."""
 import numpy as np
 import pytest
 
@@ -69,3 +70,32 @@ def test_no_gradient_follows_a_forward_pass_that_was_refused(lbm, entry):
         net.gradient(ts)
         net.close()
         assert h.live == {}
+
+
+@pytest.mark.parametrize("reason", ["zero", "negative", "nan", "timeout"])
+@pytest.mark.parametrize("entry", ["gradient", "train_step"])
+def test_a_refused_gradient_keeps_the_gradients_and_parameters(lbm, reason, entry):
+    import torch
+    x, t = _volumes(3)
+    net = lbm.Net(3, 6, 4, seed=6)
+    net.train_step(x, t)
+    grads, params = net.grads(), net.params()
+    assert np.isfinite(grads).all() and np.abs(grads).max() > 0.0
+    weight = {"zero": 0.0, "negative": -1.0, "nan": float("nan"), "timeout": 1.0}[reason] * torch.ones(x.shape[:-1], device="cuda")
+    net.forward(x)
+    net.set_wait_test(reason == "timeout")
+    with pytest.raises(lbm.LBMError) as e:
+        net.gradient(t, weight=weight) if entry == "gradient" else net.train_step(x, t, weight=weight)
+    assert e.value.status == (lbm.LBM_ETIMEOUT if reason == "timeout" else lbm.LBM_EINVAL)
+    net.set_wait_test(False)
+    assert np.array_equal(net.grads(), grads) and np.array_equal(net.params(), params)
+    # and the next gradient is that of a net with the same parameters (sums of 648 voxels in another order)
+    ref = lbm.Net(3, 6, 4, seed=6)
+    ref.set_params(params)
+    out = []
+    for n in (net, ref):
+        n.forward(x)
+        out.append((n.gradient(t), n.grads()))
+        n.close()
+    assert out[0][0] == pytest.approx(out[1][0], rel=1e-12)
+    assert np.abs(out[0][1] - out[1][1]).max() <= 648 * 2.0 ** -23 * np.abs(out[1][1]).max()
