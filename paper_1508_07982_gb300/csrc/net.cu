@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) conv_kernel(const __nv_bfloat16* __restri
 // 512 volumes of 18^3, one layer: 150 us with one MMA per tap and whole planes staged three times, now 107 (tensor
 // pipe's operand reads 83 % of the active time).
 constexpr int TC_W_BYTES = TAPS * 2 * CH * 8 * 2;   // weights [dz, dy][half][dx = 1, 0, -1][n][8] BF16
-constexpr int TC_BAR_OFF = TC_W_BYTES;              // two mbarriers, the TMEM address, a flag, the bias
+constexpr int TC_BAR_OFF = TC_W_BYTES;              // two mbarriers, the TMEM address, two flags, the bias
 constexpr int TC_TM_OFF = TC_W_BYTES + 16;
 constexpr int TC_FAIL_OFF = TC_W_BYTES + 20;
 constexpr int TC_BIAS_OFF = TC_W_BYTES + 32;
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(TC_THREADS, 3) conv_tc_kernel(const __nv_bfloa
     if (tid < CH) reinterpret_cast<float*>(sm + TC_BIAS_OFF)[tid] = bias ? bias[tid] : 0.f;
     volatile int* fail = reinterpret_cast<volatile int*>(sm + TC_FAIL_OFF);
     if (tid == 0) {
-        *fail = 0;
+        fail[0] = fail[1] = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
     }
@@ -248,12 +248,15 @@ __global__ void __launch_bounds__(TC_THREADS, 3) conv_tc_kernel(const __nv_bfloa
                     "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
                     : "=r"(done) : "r"(bar + 8 * h), "r"(phase[h]) : "memory");
             phase[h] ^= 1u;
+            // A flag per buffer: the last two drains of a unit follow one another without a barrier of the CTA between
+            // them, and a warp that reads the first one's flag late must not see what the second one set, leave, and
+            // keep the others at their barrier.
             if (!done) {
-                *fail = 1;
+                fail[h] = 1;
                 atomicExch(err, 1);
             }
             asm volatile("bar.sync 1, 128;" ::: "memory");   // the four warps agree
-            if (*fail) {
+            if (fail[h]) {
                 failed = true;
                 return;
             }
