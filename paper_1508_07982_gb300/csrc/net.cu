@@ -1093,10 +1093,11 @@ struct Coarse {
 // axis by axis over the plane: the coarse cells under it at its z (two values each, in FP64), those at each voxel
 // row's y, then the voxels along x.  FP64 operations bound the kernel, at 1.7 a clock and SM: with eight corners and
 // all spheres per voxel it took 100 a voxel (512 volumes of 18^3 at level 1: 834 us), axis by axis 20 (279 us).  Now
-// the passes along y and x run in 64-bit integers (see `fixed`), no division is left, and FP32 decides on a sphere
-// wherever its error allows, which leaves the z pass: 114 us.  Spheres whose box distance to the plane exceeds their
-// radius are left out before the voxels test them.  128 threads: the passes of a plane of 18^2 are 121, 198 and 324
-// items long and end in barriers (256 threads 114 us, 192 99, 128 and 96 85).
+// the passes along y and x run in integers that keep every bit (see `fixed`), no division is left, and FP32 decides on a
+// sphere wherever its error allows, which leaves the z pass: 95 us (85 with 64-bit integers alone, which cut values far
+// below the plane's largest).  Spheres whose box distance to the plane exceeds their radius are left out before the
+// voxels test them.  128 threads: the passes of a plane of 18^2 are 121, 198 and 324 items long and end in barriers
+// (64-bit integers, 256 threads: 114 us, 192 99, 128 and 96 85).
 constexpr int kFeatThreads = 128;
 constexpr int kFeatSpheres = 64;   // spheres tested per round
 constexpr int kFeatTile = 32;
@@ -1111,7 +1112,7 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(Coarse c, int le
     __shared__ int nnear;
     __shared__ int wgt[2][kFeatTile];       // weight of the upper coarse cell along x and y, of 2^(L + 1)
     __shared__ int at[2][kFeatTile];        // the lower coarse cell, from the part's first
-    __shared__ int top[4];                  // the largest exponent of each component on the plane
+    __shared__ int top[4], low[4];          // the largest exponent of each component on the plane, and of its non-zero values the smallest
     __shared__ double wz[4];                // weights along z times the scales: density lower, upper, velocity lower, upper
     const int D = B + 2 * halo;
     const int tile = int(blockIdx.x % unsigned(nt * nt));
@@ -1132,20 +1133,26 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(Coarse c, int le
         at[a][i] = cell(g0[a] + i) - (a == 0 ? cx0 : cy0);
     }
     const int ncx = cell(g0[0] + TX - 1) - cx0 + 2, ncy = cell(g0[1] + TY - 1) - cy0 + 2;
-    long long* const plane = fsm;                    // [4][ncy][ncx] at the plane's z: bits of doubles, or whole numbers
-    long long* const rows = fsm + 4 * ncx * ncy;     // [4][TY][ncx] at each voxel row's y
+    // at the plane's z [4][ncy][ncx], and at each voxel row's y [4][TY][ncx]: bits of doubles, or the upper limbs of
+    // whole numbers, whose lower limbs lie behind
+    const int np = ncx * ncy, nr = TY * ncx;
+    long long* const plane = fsm;
+    long long* const rows = plane + 4 * np;
+    uint32_t* const plane_lo = reinterpret_cast<uint32_t*>(rows + 4 * nr);
+    uint32_t* const rows_lo = plane_lo + 4 * np;
     // i / ncx and i / TX for i < 34^2 (i times the reciprocal's error stays below 2^16)
     const unsigned by_ncx = (65535u + unsigned(ncx)) / unsigned(ncx), by_tx = (65535u + unsigned(TX)) / unsigned(TX);
     const int gz = g0[2] + vz, cz = cell(gz);
     if (tid < 4) {
         top[tid] = 0;
+        low[tid] = 0x7FF;
         const int w1 = weight(gz);
         wz[tid] = double(tid & 1 ? w1 : (2 << level) - w1) * wunit * (tid < 2 ? rho_scale : u_scale);
     }
     __syncthreads();
     {
-        int e[4] = {0, 0, 0, 0};
-        for (int i = tid; i < ncx * ncy; i += kFeatThreads) {
+        int e[4] = {0, 0, 0, 0}, m[4] = {0x7FF, 0x7FF, 0x7FF, 0x7FF};
+        for (int i = tid; i < np; i += kFeatThreads) {
             const int j = int((unsigned(i) * by_ncx) >> 16);
             double v[2][4];
 #pragma unroll
@@ -1161,56 +1168,79 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(Coarse c, int le
 #pragma unroll
             for (int a = 0; a < 4; a++) {
                 const long long t = __double_as_longlong(wz[a ? 2 : 0] * v[0][a] + wz[a ? 3 : 1] * v[1][a]);
-                plane[a * ncx * ncy + i] = t;
-                // a zero leaves the exponent at 0, so that a component of zeros has none
-                e[a] = max(e[a], (t << 1) == 0 ? 0 : max(int(t >> 52) & 0x7FF, 1));
+                plane[a * np + i] = t;
+                const int x = max(int(t >> 52) & 0x7FF, 1);
+                if (t << 1) {   // a component of zeros has no exponent
+                    e[a] = max(e[a], x);
+                    m[a] = min(m[a], x);
+                }
             }
         }
 #pragma unroll
         for (int a = 0; a < 4; a++) {
-            const int m = __reduce_max_sync(0xFFFFFFFFu, e[a]);
-            if ((tid & 31) == 0 && m > 0) atomicMax(&top[a], m);
+            const int hi = __reduce_max_sync(0xFFFFFFFFu, e[a]), lo = __reduce_min_sync(0xFFFFFFFFu, m[a]);
+            if ((tid & 31) == 0 && hi > 0) {
+                atomicMax(&top[a], hi);
+                atomicMin(&low[a], lo);
+            }
         }
     }
     __syncthreads();
-    // The weights along y and x are whole numbers of 2^(L + 1)ths, so these two passes run in 64-bit integers: a
-    // plane's component is scaled by the power of two that puts its largest value just below 2^bits, which leaves room
-    // for both weights and, up to level 3, every bit of that value.  bits >= 54: the rounding is 2^-54 of the plane's
-    // largest value at most, half of what FP64 rounds it by.  back: the power of two to a float.
+    // The weights along y and x are whole numbers of 2^(L + 1)ths, so these two passes run in integers of an upper limb
+    // of 64 bits and a lower one of 32: a plane's component is scaled by the power of two that puts its largest value
+    // just below 2^(bits + 32), which leaves room for both weights.  Every bit of every value is kept, so that the float
+    // is the only rounding (FP64 sums round each term to 2^-53), where the component's smallest value is not too far
+    // below its largest (2^-39 of it at level 0, 2^-33 at level 3); other planes take FP64.  back: the power of two to a float,
+    // with 2^-32 for the values that the lower limb reaches still in the normal range.
     const int bits = 62 - 2 * (level + 1);
     bool fixed = level <= 3;
     float back[4];
 #pragma unroll
     for (int a = 0; a < 4; a++) {
         const int t = top[a] - 1022 - 62;
-        if (top[a] != 0 && (t < -126 || t > 127)) fixed = false;   // infinities and NaN; scales beyond a float's
+        // infinities and NaN, scales beyond a float's, values that would lose bits
+        if (top[a] != 0 && (t < -118 || t > 127 || top[a] - low[a] > bits + 32 - 53)) fixed = false;
         back[a] = top[a] == 0 || !fixed ? 0.f : __int_as_float((t + 127) << 23);
     }
     if (fixed) {
-        for (int i = tid; i < ncx * ncy; i += kFeatThreads)
+        for (int i = tid; i < np; i += kFeatThreads)
 #pragma unroll
             for (int a = 0; a < 4; a++) {
-                const long long v = plane[a * ncx * ncy + i];
+                const long long v = plane[a * np + i];
                 const int e = int(v >> 52) & 0x7FF;
-                const long long m = (v & 0xFFFFFFFFFFFFFLL) | (e ? 1LL << 52 : 0LL);
-                const int sh = bits - 53 - (top[a] - max(e, 1));
-                const long long q = sh >= 0 ? m << sh : sh < -54 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
-                plane[a * ncx * ncy + i] = v < 0 ? -q : q;
+                const unsigned long long m = (unsigned long long)(v & 0xFFFFFFFFFFFFFLL) | (e ? 1ULL << 52 : 0ULL);
+                const int sh = m ? bits + 32 - 53 - (top[a] - max(e, 1)) : 0;   // 0 to 39
+                long long hi = (long long)(sh < 32 ? m >> (32 - sh) : m << (sh - 32));
+                uint32_t lo = sh < 32 ? uint32_t(m) << sh : 0u;
+                if (v < 0) {   // the two's complement of both limbs
+                    lo = 0u - lo;
+                    hi = -hi - (lo != 0u);
+                }
+                plane[a * np + i] = hi;
+                plane_lo[a * np + i] = lo;
             }
         __syncthreads();
     }
-    for (int i = tid; i < TY * ncx; i += kFeatThreads) {
+    // w0 p + w1 q of two numbers, the lower limb's carry added
+    auto mix = [](int w0, int w1, long long ph, uint32_t pl, long long qh, uint32_t ql, uint32_t& lo) {
+        const unsigned long long l = (unsigned long long)(pl) * unsigned(w0) + (unsigned long long)(ql) * unsigned(w1);
+        lo = uint32_t(l);
+        return w0 * ph + w1 * qh + (long long)(l >> 32);
+    };
+    for (int i = tid; i < nr; i += kFeatThreads) {
         const int y = int((unsigned(i) * by_ncx) >> 16), cx = i - y * ncx;
         const int w1 = wgt[1][y], w0 = (2 << level) - w1, o = at[1][y] * ncx + cx;
         if (fixed) {
 #pragma unroll
-            for (int a = 0; a < 4; a++)
-                rows[a * TY * ncx + i] = w0 * plane[a * ncx * ncy + o] + w1 * plane[a * ncx * ncy + o + ncx];
+            for (int a = 0; a < 4; a++) {
+                const int p = a * np + o;
+                rows[a * nr + i] = mix(w0, w1, plane[p], plane_lo[p], plane[p + ncx], plane_lo[p + ncx], rows_lo[a * nr + i]);
+            }
         } else {
 #pragma unroll
             for (int a = 0; a < 4; a++)
-                rows[a * TY * ncx + i] = __double_as_longlong(w0 * wunit * __longlong_as_double(plane[a * ncx * ncy + o]) +
-                                                              w1 * wunit * __longlong_as_double(plane[a * ncx * ncy + o + ncx]));
+                rows[a * nr + i] = __double_as_longlong(w0 * wunit * __longlong_as_double(plane[a * np + o]) +
+                                                        w1 * wunit * __longlong_as_double(plane[a * np + o + ncx]));
         }
     }
     const float sf = __int_as_float((127 - level) << 23);   // 2^-L
@@ -1277,13 +1307,21 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(Coarse c, int le
             float f[4];
             if (fixed) {
 #pragma unroll
-                for (int a = 0; a < 4; a++)
-                    f[a] = __ll2float_rn(w0 * rows[a * TY * ncx + o] + w1 * rows[a * TY * ncx + o + 1]) * back[a];
+                for (int a = 0; a < 4; a++) {
+                    const int p = a * nr + o;
+                    uint32_t lo;
+                    const long long hi = mix(w0, w1, rows[p], rows_lo[p], rows[p + 1], rows_lo[p + 1], lo);
+                    // one rounding to 24 bits: of both limbs where they fit in 64 bits, else of the upper one with a
+                    // last bit for what lies below it
+                    const bool both = (unsigned long long)(hi + (1LL << 30)) < (1ULL << 31);
+                    const long long t = both ? (long long)((unsigned long long)(hi) << 32 | lo) : hi | (lo != 0u);
+                    f[a] = __ll2float_rn(t) * (both ? 0x1p-32f : 1.f) * back[a];
+                }
             } else {
 #pragma unroll
                 for (int a = 0; a < 4; a++)
-                    f[a] = float(w0 * wunit * __longlong_as_double(rows[a * TY * ncx + o]) +
-                                 w1 * wunit * __longlong_as_double(rows[a * TY * ncx + o + 1]));
+                    f[a] = float(w0 * wunit * __longlong_as_double(rows[a * nr + o]) +
+                                 w1 * wunit * __longlong_as_double(rows[a * nr + o + 1]));
             }
             const float flag = solid ? 1.f : 0.f, lev = float(level) * 0.5f;
             if (wide) {
@@ -1370,10 +1408,10 @@ lbm_status lbm_warmstart_features(const double* coarse_rho, const double* coarse
     const long long ctas = (long long)D * nblocks * nt * nt;
     if (ctas >= (1LL << 31)) return nfail(LBM_EINVAL, "too many volumes");
     // the coarse cells under T voxels of an axis: at most (T - 1) / 2^level + 1 of them and the upper neighbour, which
-    // at kFeatTile and level 0 take 72 KB
+    // at kFeatTile and level 0 take 108 KB
     const int nc = (T - 1) / (1 << level) + 3;
-    const size_t smem = size_t(4) * (nc * nc + T * nc) * sizeof(double);
-    NCU(cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024));
+    const size_t smem = size_t(4) * (nc * nc + T * nc) * (sizeof(long long) + sizeof(uint32_t));
+    NCU(cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));
     features_kernel<<<unsigned(ctas), kFeatThreads, smem, static_cast<cudaStream_t>(stream)>>>(
         c, level, B, halo, blocks, spheres, nspheres, rho_scale, u_scale, T, nt, static_cast<__nv_bfloat16*>(x), skip);
     NCU(cudaGetLastError());
