@@ -330,8 +330,8 @@ def _uniform(case):
 
 def _batch(lbm, torch, steps=500, warmup=5, serial_steps=50):
     """The batched workload: 256 small lid-driven cavities (2-3 levels, 16^3 blocks, 8-64 leaves
-    each) stepped together, one launch per phase, after autotuning the batch's thread mapping;
-    beside it the same members stepped one forest after another."""
+    each) stepped together, one launch per phase; beside it the same members stepped one forest after
+    another."""
     from paper_1508_07982_gb300 import inputs
     cases = inputs.batch_cases()
     fs = []
@@ -340,7 +340,6 @@ def _batch(lbm, torch, steps=500, warmup=5, serial_steps=50):
         f.init_uniform()
         fs.append(f)
     b = lbm.Batch(fs)
-    lzc, minb, _ = b.autotune(4)
     b.step(warmup)
     torch.cuda.synchronize()
     stream = torch.cuda.current_stream()
@@ -369,7 +368,6 @@ def _batch(lbm, torch, steps=500, warmup=5, serial_steps=50):
            "value": round(upd * steps / (ms / 1e3) / 1e9, 4), "unit": UNIT, "precision": "fp32s",
            "steps": steps, "warmup": warmup, "ms_per_step": round(ms / steps, 5),
            "cell_updates_per_coarse_step": int(upd), "gpu_launches_per_coarse_step": int(launches),
-           "kernel_config": {"cells_per_thread_log2": lzc, "ctas_per_sm": minb},
            "one_forest_at_a_time": {"value": round(upd * serial_steps / (ms_serial / 1e3) / 1e9, 4), "unit": UNIT,
                                     "ms_per_step": round(ms_serial / serial_steps, 5), "steps": serial_steps}}
     b.close()

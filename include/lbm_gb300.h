@@ -255,9 +255,9 @@ lbm_status lbm_timing_end(lbm_forest* f, double* ms_per_level, int64_t* launches
                           double* ms_side_per_level, int64_t* launches_side_per_level);
 
 /* Launch configuration of the stream-collide kernel (results do not depend on it).  The kernels
- * have one mapping for each storage type (the fastest of 2 to 5 CTAs per SM on the sphere channel):
- * four x-adjacent cells per lane and 3 (LBM_FP32S) or 4 (LBM_FP16S) resident 128-thread CTAs per
- * SM; one cell per thread and 4 CTAs per SM for LBM_FP64.  So the call checks its arguments
+ * have one mapping for each storage type (the fastest of those tried on the sphere channel): four
+ * x-adjacent cells per lane and 6 (LBM_FP32S) or 8 (LBM_FP16S) resident CTAs of 64 threads per SM;
+ * one cell per thread and 4 CTAs of 128 threads per SM for LBM_FP64.  So the call checks its arguments
  * (2^cells_per_thread_log2 <= B, ctas_per_sm 1 to 4) and keeps them for lbm_get_kernel_config, but
  * launches do not change with them.  The default is (log2 B - 3, 3) for LBM_FP64 and
  * (log2 B - 3, 2) otherwise.  Synchronises the stream and drops the captured graphs; the next
@@ -268,21 +268,22 @@ lbm_status lbm_get_kernel_config(const lbm_forest* f, int32_t* cells_per_thread_
 /* Number of kernel launches one coarse step issues (the nodes of the captured graph). */
 lbm_status lbm_launches_per_coarse_step(const lbm_forest* f, int32_t* n);
 
-/* Picks the fastest thread mapping for this forest: times n_steps coarse steps (Alg. 1) for every
- * (cells_per_thread_log2 <= log2 B, ctas_per_sm in 1..4) pair, applies the fastest as
- * lbm_set_kernel_config would, and writes it and its ms per coarse step (outputs may be NULL).
+/* Times this forest: n_steps coarse steps (Alg. 1) after two that are not timed, ms per coarse step to
+ * *ms_per_step.  The kernels have one thread mapping for each storage type, so there is nothing to
+ * choose: the launch configuration stays as set (lbm_set_kernel_config) and is written to the other
+ * two outputs (any may be NULL).
  * The state of the forest (every level's two PDF grids and parities) is copied on the device first
  * and restored afterwards, so the call leaves the simulation where it was; the copy needs as much
- * device memory again as the PDF grids.  The results of later steps do not depend on the mapping.
- * Synchronises the stream.  LBM_EINVAL if the forest is not initialised or is being timed. */
+ * device memory again as the PDF grids.  Synchronises the stream.  LBM_EINVAL if the forest is not
+ * initialised or is being timed. */
 lbm_status lbm_autotune(lbm_forest* f, int32_t n_steps, int32_t* cells_per_thread_log2, int32_t* ctas_per_sm,
                         double* ms_per_step);
 
 /* Picks the block size for a description: for every B in {8, 16, 32} that divides the domain
  * (root_blocks x block_cells level-0 cells per axis, kept fixed: root_blocks becomes N / B) it
  * creates the forest with block size B (through `alloc`, on `stream`), sets the level parameters as
- * lbm_set_level_params(lambda_e0, magic_lambda, accel0) does, starts it from rest, tunes its thread
- * mapping as lbm_autotune(n_steps) does, and destroys it; it writes the B with the fewest ms per
+ * lbm_set_level_params(lambda_e0, magic_lambda, accel0) does, starts it from rest, times it as
+ * lbm_autotune(n_steps) does, and destroys it; it writes the B with the fewest ms per
  * coarse step to *block_cells and each candidate's ms to ms_per_step[0..2] (B = 8, 16, 32; -1 where
  * B does not divide the domain or the forest cannot be built).  The regions and obstacles are the
  * same for every B, but refinement splits whole blocks, so a larger B covers the requested regions
@@ -310,9 +311,9 @@ lbm_status lbm_autotune_block_size(const lbm_forest_desc* d, lbm_refine_fn refin
  * its graphs, so it must be destroyed and re-created after a member is re-created.
  * lbm_batch_step(b, n): n coarse steps of every member on the members' stream (graph replay,
  * asynchronous); every member must be initialised, with parameters set, and at the same two-grid
- * parity (members stepped only together are).  lbm_batch_set_kernel_config / lbm_batch_autotune
- * set or tune the thread mapping of the batch's launches as the single-forest calls do (autotune
- * restores every member's state).  lbm_batch_cell_updates_per_coarse_step sums the members' cell
+ * parity (members stepped only together are).  lbm_batch_set_kernel_config checks and keeps a
+ * launch configuration, and lbm_batch_autotune times the batch and restores every member's state, as
+ * the single-forest calls do.  lbm_batch_cell_updates_per_coarse_step sums the members' cell
  * updates; lbm_batch_launches_per_coarse_step counts the launches of one coarse step. */
 typedef struct lbm_batch lbm_batch;
 lbm_status lbm_batch_create(lbm_forest* const* forests, int32_t n, const lbm_allocator* alloc,

@@ -228,7 +228,7 @@ struct lbm_forest {
     int tmax = 0, tused = 0;
     std::vector<cudaEvent_t> tev;
     int64_t updates = 0;
-    int lzc = 3, minb = 3;   // the launch configuration set or tuned (the kernels have one mapping)
+    int lzc = 3, minb = 3;   // the launch configuration as set (the kernels have one mapping)
     std::vector<int64_t> tot_warps;   // per level: warp entries its recording launch writes
     bool totals_valid = false;        // the recorded moments describe the current state
     std::vector<double*> uprev;   // per level, the velocity of the previous residual call
@@ -1125,7 +1125,7 @@ lbm_status lbm_timing_end(lbm_forest* f, double* ms_per_level, int64_t* launches
 
 }  // extern "C"
 
-// ------------------------------------------------------------------ kernel-config autotuning
+// ------------------------------------------------------------------ autotuning
 namespace {
 
 // Device copy of every level's two PDF grids and the parities, so that tuning runs leave the
@@ -1174,11 +1174,10 @@ void free_snapshot(Snapshot& sn) {
     sn.owner.clear();
 }
 
-// Times n_steps of `step` for every (cells per thread, CTAs per SM) the kernels support and
-// keeps the fastest; `config` applies one.  Results do not depend on the configuration.
-template <typename Config, typename Step>
-lbm_status tune(const std::vector<lbm_forest*>& fs, cudaStream_t s, int LB, int n_steps, Config config, Step step,
-                int32_t* best_lzc, int32_t* best_minb, double* best_ms) {
+// ms per call of `step` over n_steps of them, after two that capture the graphs of both parities; the state is put
+// back.  The kernels have one mapping, so one run serves every launch configuration.
+template <typename Step>
+lbm_status tune(const std::vector<lbm_forest*>& fs, cudaStream_t s, int n_steps, Step step, double* ms_per_step) {
     Snapshot sn;
     lbm_status st = take_snapshot(fs, s, sn);
     if (st) {
@@ -1186,24 +1185,14 @@ lbm_status tune(const std::vector<lbm_forest*>& fs, cudaStream_t s, int LB, int 
         return st;
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    double best = 1e300;
-    int bl = LB - 3 > 0 ? LB - 3 : 0, bm = 3;
+    float ms = 0.f;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) st = fail(LBM_ECUDA, "cudaEventCreate failed");
-    for (int lzc = 0; lzc <= LB && !st; lzc++)
-        for (int minb = 1; minb <= 4 && !st; minb++) {
-            if ((st = config(lzc, minb)) || (st = step(1))) break;   // the first step captures the graphs
-            if (cudaEventRecord(e0, s) != cudaSuccess) st = fail(LBM_ECUDA, "cudaEventRecord failed");
-            if (!st) st = step(n_steps);
-            if (!st && cudaEventRecord(e1, s) != cudaSuccess) st = fail(LBM_ECUDA, "cudaEventRecord failed");
-            float ms = 0.f;
-            if (!st && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-                st = fail(LBM_ECUDA, "timing a configuration failed");
-            if (!st && ms / n_steps < best) {
-                best = ms / n_steps;
-                bl = lzc;
-                bm = minb;
-            }
-        }
+    if (!st) st = step(2);
+    if (!st && cudaEventRecord(e0, s) != cudaSuccess) st = fail(LBM_ECUDA, "cudaEventRecord failed");
+    if (!st) st = step(n_steps);
+    if (!st && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+        st = fail(LBM_ECUDA, "timing the steps failed");
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     lbm_status rs = restore_snapshot(fs, s, sn);
@@ -1211,10 +1200,7 @@ lbm_status tune(const std::vector<lbm_forest*>& fs, cudaStream_t s, int LB, int 
     free_snapshot(sn);
     if (st) return st;
     if (rs) return rs;
-    if ((st = config(bl, bm))) return st;
-    if (best_lzc) *best_lzc = bl;
-    if (best_minb) *best_minb = bm;
-    if (best_ms) *best_ms = best;
+    if (ms_per_step) *ms_per_step = double(ms) / n_steps;
     return LBM_OK;
 }
 
@@ -1226,9 +1212,11 @@ extern "C" lbm_status lbm_autotune(lbm_forest* f, int32_t n_steps, int32_t* cell
     if (!f->params_set || f->init_mask != (1u << f->plan.nlev) - 1)
         return fail(LBM_EINVAL, "set the level parameters and initialise every level before tuning");
     if (f->timing) return fail(LBM_EINVAL, "timing is active");
-    return tune(
-        {f}, f->stream, f->plan.LB, n_steps, [&](int l, int m) { return lbm_set_kernel_config(f, l, m); },
-        [&](int n) { return lbm_step_coarse(f, n); }, cells_per_thread_log2, ctas_per_sm, ms_per_step);
+    const lbm_status st = tune({f}, f->stream, n_steps, [&](int n) { return lbm_step_coarse(f, n); }, ms_per_step);
+    if (st) return st;
+    if (cells_per_thread_log2) *cells_per_thread_log2 = f->lzc;
+    if (ctas_per_sm) *ctas_per_sm = f->minb;
+    return LBM_OK;
 }
 
 extern "C" lbm_status lbm_autotune_block_size(const lbm_forest_desc* d, lbm_refine_fn refine, lbm_flag_fn flag,
@@ -1290,7 +1278,7 @@ struct lbm_batch {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     const Launchers* L = nullptr;
     int nlev = 0, LB = 0, collision = 0;
-    int lzc = 2, minb = 3;   // the launch configuration set or tuned (the kernels have one mapping)
+    int lzc = 2, minb = 3;   // the launch configuration as set (the kernels have one mapping)
     std::vector<BatchPhase> phases;
     cudaGraphExec_t exec[2] = {};
     int64_t updates = 0;
@@ -1572,9 +1560,11 @@ lbm_status lbm_batch_launches_per_coarse_step(const lbm_batch* b, int32_t* n) {
 lbm_status lbm_batch_autotune(lbm_batch* b, int32_t n_steps, int32_t* cells_per_thread_log2, int32_t* ctas_per_sm,
                               double* ms_per_step) {
     if (!b || n_steps < 1) return fail(LBM_EINVAL, "invalid argument");
-    return tune(
-        b->fs, b->stream, b->LB, n_steps, [&](int l, int m) { return lbm_batch_set_kernel_config(b, l, m); },
-        [&](int n) { return lbm_batch_step(b, n); }, cells_per_thread_log2, ctas_per_sm, ms_per_step);
+    const lbm_status st = tune(b->fs, b->stream, n_steps, [&](int n) { return lbm_batch_step(b, n); }, ms_per_step);
+    if (st) return st;
+    if (cells_per_thread_log2) *cells_per_thread_log2 = b->lzc;
+    if (ctas_per_sm) *ctas_per_sm = b->minb;
+    return LBM_OK;
 }
 
 }  // extern "C"

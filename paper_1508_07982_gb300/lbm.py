@@ -491,8 +491,8 @@ class Forest:
         return a.value, b.value
 
     def autotune(self, n_steps=10):
-        """lbm_autotune: applies the fastest thread mapping; returns (cells_per_thread_log2,
-        ctas_per_sm, ms per coarse step).  The state is left as it was."""
+        """lbm_autotune: times n_steps; returns the launch configuration as set (cells_per_thread_log2,
+        ctas_per_sm) and the ms per coarse step.  The state is left as it was."""
         a, b, ms = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_double()
         _check(library().lbm_autotune(self.h, n_steps, ctypes.byref(a), ctypes.byref(b), ctypes.byref(ms)))
         return a.value, b.value, ms.value
