@@ -61,7 +61,7 @@ struct Launch {
 struct DevBuf {
     void* f[2] = {nullptr, nullptr};
     uint8_t* cell = nullptr;
-    int32_t *nbr = nullptr, *parent = nullptr, *child = nullptr, *pos = nullptr;
+    int32_t *nbr = nullptr, *parent = nullptr, *pos = nullptr;
     uint32_t* link = nullptr;
     uint32_t *gcopy[2] = {nullptr, nullptr}, *gseg[2] = {nullptr, nullptr}, *gspec[2] = {nullptr, nullptr};
     uint32_t *ecopy = nullptr, *eseg = nullptr;
@@ -597,7 +597,6 @@ lbm_status lbm_destroy(lbm_forest* f) {
         m.put(b.cell);
         m.put(b.nbr);
         m.put(b.parent);
-        m.put(b.child);
         m.put(b.pos);
         m.put(b.link);
         for (int s = 0; s < 2; s++)
@@ -675,8 +674,8 @@ lbm_status lbm_create_forest(const lbm_forest_desc* d, lbm_refine_fn refine, lbm
         std::vector<int32_t> nbr(V.nbr);   // the centre entries hold the bricks' attributes
         for (int k = 0; k < V.nbricks(); k++) nbr[size_t(k) * 27 + 13] = V.kind[k];
         if ((s = upload(m, &b.cell, V.cell)) || (s = upload(m, &b.nbr, nbr)) || (s = upload(m, &b.parent, V.parent)) ||
-            (s = upload(m, &b.child, V.child)) || (s = upload(m, &b.pos, V.pos)) || (s = upload(m, &b.link, V.link)) || (s = upload(m, &b.ecopy, V.ecopy)) || (s = upload(m, &b.eseg, V.eseg)) ||
-            (s = upload(m, &b.cwork, V.cwork)))
+            (s = upload(m, &b.pos, V.pos)) || (s = upload(m, &b.link, V.link)) || (s = upload(m, &b.ecopy, V.ecopy)) ||
+            (s = upload(m, &b.eseg, V.eseg)) || (s = upload(m, &b.cwork, V.cwork)))
             return bail(s);
         for (int k = 0; k < 2; k++)
             if ((s = upload(m, &b.gcopy[k], V.gcopy[k])) || (s = upload(m, &b.gseg[k], V.gseg[k])) ||
@@ -693,7 +692,6 @@ lbm_status lbm_create_forest(const lbm_forest_desc* d, lbm_refine_fn refine, lbm
         g.cell = b.cell;
         g.nbr = b.nbr;
         g.parent = b.parent;
-        g.child = b.child;
         g.pos = b.pos;
         g.link = b.link;
         g.ecopy = reinterpret_cast<const uint2*>(b.ecopy);

@@ -41,7 +41,6 @@ struct DevLevel {
     const uint8_t* cell;  // [ncells] CK_*
     const int32_t* nbr;   // [nbricks][27], the centre entry holding the brick's BK_* bits
     const int32_t* parent;
-    const int32_t* child;
     const int32_t* pos;   // [nbricks][3]
     const uint32_t* link;    // [nown * B^3] per owned cell: bit q set = link q needs the general
                              // pull; bits 25-27 and 29 bounce-back; bit 30 = a coupled cell;
