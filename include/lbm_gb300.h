@@ -367,7 +367,11 @@ lbm_status lbm_probe_fp64_fma(int32_t reps, double* gfma, void* stream);
  * 0.999, eps 1e-8) with learning rate lr.  All pointers except the host parameter buffers are
  * device pointers; calls run on `stream` and synchronise it where they return a loss.  The
  * parameters, optimiser moments and the activations of the largest volume set seen so far come
- * from `alloc` (NULL: cudaMalloc); a call on more voxels than before grows the activations. */
+ * from `alloc` (NULL: cudaMalloc); a call on more voxels than before grows the activations.
+ * After a forward or predict call that was refused (LBM_ENOMEM) lbm_net_gradient returns LBM_EINVAL
+ * until another one is accepted.  A gradient or training call that is refused (loss weights without a
+ * positive sum, LBM_EINVAL) or times out (LBM_ETIMEOUT) leaves the parameters and the gradients of
+ * the last accepted one as they are. */
 typedef struct lbm_net lbm_net;
 
 /* Data movement of the warm start (device pointers, asynchronous on `stream`).
@@ -409,17 +413,16 @@ lbm_status lbm_net_gradient(lbm_net* n, const float* skip, const float* target, 
 lbm_status lbm_net_get_grads(const lbm_net* n, float* host);
 lbm_status lbm_net_train_step(lbm_net* n, const void* x, const float* skip, const float* target, const float* weight,
                               int32_t D, int32_t H, int32_t W, int32_t nvol, float lr, double* loss);
-/* Tensor-core path of the convolutions: 1 (default) runs them with tcgen05.mma into TMEM where
- * a volume's zero-padded planes fit in shared memory (W, H up to about 40), 0 with warp-level
- * mma.sync everywhere.  Both compute the same products in BF16 x BF16 -> FP32; the sums are
- * ordered differently.  Calls that wait on the tcgen05 kernel return LBM_ETIMEOUT if one of its
+/* Tensor-core path of the convolutions: 1 (default) runs them with tcgen05.mma into TMEM (planes of
+ * fewer than 2^29 voxels, larger ones with mma.sync), 0 with warp-level mma.sync everywhere.  Both
+ * compute the same products in BF16 x BF16 -> FP32; the sums are ordered differently.  Calls that wait on the tcgen05 kernel return LBM_ETIMEOUT if one of its
  * bounded waits ran out. */
 lbm_status lbm_net_set_backend(lbm_net* n, int32_t backend);
 /* Test of the timeout path: with on = 1 the tcgen05 convolution issues no tensor-core products and
  * polls its mbarrier at most 1,024 times, so the wait runs out with nothing asynchronous in flight;
  * the kernel flags it, releases its tensor memory and returns, and the call that waits on it
- * (lbm_net_forward, lbm_net_predict, lbm_net_train_step) returns LBM_ETIMEOUT with incomplete
- * outputs.  on = 0 (the default) restores normal operation.  No GPU fault is involved. */
+ * (lbm_net_forward, lbm_net_predict, lbm_net_gradient, lbm_net_train_step) returns LBM_ETIMEOUT with
+ * incomplete outputs.  on = 0 (the default) restores normal operation.  No GPU fault is involved. */
 lbm_status lbm_net_set_wait_test(lbm_net* n, int32_t on);
 
 /* ---- totals without allocation ------------------------------------------------------------

@@ -5,7 +5,8 @@
 // Net: L layers of 3x3x3 convolutions (zero padding, stride 1), width 16, ReLU between layers,
 // none after the last.  Tensors are channels-last volumes of 16 BF16 channels (32 bytes per
 // voxel), `nvol` volumes of D x H x W voxels stored one after another, x fastest.  Products
-// run on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulate).  Weights are kept
+// run on the tensor cores (BF16 operands, FP32 accumulate): the convolutions with tcgen05.mma, or with
+// mma.sync m16n8k16 where the caller asks for it, the weight gradient with mma.sync.  Weights are kept
 // in FP32 (master copy, Adam moments) and rounded to BF16 for the products.
 //
 //   forward   Z_l = b_l + sum_o W_l[o] X_l[v + o]          X_{l+1} = relu(Z_l)
@@ -121,8 +122,10 @@ __global__ void __launch_bounds__(256) conv_kernel(const __nv_bfloat16* __restri
 // While plane z multiplies (one thread of a warp of its own issues, about as long as the products take; FP32
 // accumulators in one of two TMEM buffers, a commit to an mbarrier), four warps read plane z - 1 from the other buffer (tcgen05.ld 32x32b.x16: a voxel's 16 channels), apply bias and
 // activation as conv_kernel does and store 128 bytes per lane, and the copies of plane z + 2 are in flight.
-// 512 volumes of 18^3, one layer: 150 us with one MMA per tap and whole planes staged three times, now 107 (tensor
-// pipe's operand reads 83 % of the active time).
+// 512 volumes of 18^3, one layer: 150 us with one MMA per tap and whole planes staged three times, now 107.  Bound:
+// the shared-memory pipe, 88 % of the elapsed time (65 % the MMAs' operand reads, 23 % the copies and the bias reads,
+// two thirds of them bank conflicts), and the wait for a plane's copies with a CTA barrier: with a third of the MMAs a
+// layer still takes 85 us.
 constexpr int TC_W_BYTES = TAPS * 2 * CH * 8 * 2;   // weights [dz, dy][half][dx = 1, 0, -1][n][8] BF16
 constexpr int TC_BAR_OFF = TC_W_BYTES;              // two mbarriers, the TMEM address, two flags, the bias
 constexpr int TC_TM_OFF = TC_W_BYTES + 16;
